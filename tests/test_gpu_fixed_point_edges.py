@@ -1,0 +1,93 @@
+"""The integer-pipe kernels of the 2D path at the edges of what they take."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+KB = [(1, O.BASIS_Q), (1, O.BASIS_P), (2, O.BASIS_Q), (2, O.BASIS_P), (3, O.BASIS_Q), (3, O.BASIS_P)]
+SYSTEMS = [O.EULER, O.ADVECTION, O.BURGERS]
+
+
+def _desc(system, k, basis, nx, ny, bx=1.0, by=1.0, bc=O.PERIODIC, rk=3, gamma=1.4):
+    return dict(dim=2, nx=nx, ny=ny, k=k, basis=basis, system=system, bc=bc, oe=1, rk=rk, ax=0.0, bx=bx, ay=0.0,
+                by=by, gamma=gamma, cfl=0.1, adv_x=1.0, adv_y=-0.7)
+
+
+def _pair(*a, **kw):
+    from paper_2503_12473_gb300 import oecdg as G
+    d = _desc(*a, **kw)
+    return O.Problem(**d), G.Context(G.MeshDesc(**d))
+
+
+def _state(p, rng, size=0.02):
+    """Coefficients of the given size about a uniform physical state."""
+    u = size * rng.standard_normal(p.shape)
+    u[:, :, 0] += np.array([1.0, 0.3, -0.2, 4.0] if p.nfields == 4 else [1.0])[None, :, None, None]
+    if p.nxs != p.nx or p.nys != p.ny:  # the primal mesh leaves the padded slots at 0
+        u[0, :, :, p.ny:] = 0.0
+        u[0, :, :, :, p.nx:] = 0.0
+    return u
+
+
+SIDES = {"periodic": O.PERIODIC, "outflow": O.TRANSMISSIVE,
+         "mixed": (O.PERIODIC, O.PERIODIC, O.TRANSMISSIVE, O.TRANSMISSIVE),
+         "walls": (O.REFLECTIVE, O.TRANSMISSIVE, O.REFLECTIVE, O.REFLECTIVE)}
+
+
+@pytest.mark.parametrize("system", SYSTEMS)
+@pytest.mark.parametrize("k,basis", KB)
+def test_zeros_stay_exactly_zero(k, basis, system):
+    """A state of zeros (either sign), and an Euler state without momentum: its
+    right-hand side, damping and sigma are zeros, not the last unit of a block (a
+    field that is 0 everywhere takes no part in delta)."""
+    p, ctx = _pair(system, k, basis, 11, 6, by=0.5)
+    u = _state(p, np.random.default_rng(k))
+    if system == O.EULER:
+        u[:, 1:3] = 0.0
+        zero = [1, 2]
+    else:
+        u[:] = 0.0
+        zero = [0]
+    u[:, zero, ::2] = -0.0
+    ug = torch.from_numpy(u).cuda()
+    d = torch.zeros((2, p.ny, p.nx, p.k + 1), dtype=torch.float64, device="cuda")
+    s = torch.zeros((2, p.nfields), dtype=torch.float64, device="cuda")
+    ctx.cdg_oe_coefficients(ug, d, s)
+    ref, _, _, st = O.oe_coefficients(p, u)
+    assert st == O.OK and (s.cpu().numpy()[:, zero] == 0.0).all()
+    # differences and sigma of 0.02 from averages of 4: 100 roundings of 2^-53 x 200
+    assert np.abs(d.cpu().numpy() - ref).max() <= 3e-12 * np.abs(ref).max()
+    L, out = torch.ones_like(ug), torch.ones_like(ug)
+    ctx.cdg_rhs(ug, 1e-3, L)
+    ctx.cdg_set_dt(1e-3, 1e-3)
+    ctx.cdg_oe_damp(ug, out)
+    assert (out[:, zero] == 0.0).all()
+    if system != O.EULER:
+        assert (L == 0.0).all()
+        ctx.cdg_rk_stage(0, ug, ug, out)
+        assert (out == 0.0).all()
+
+
+def test_a_transverse_momentum_of_zero_stays_zero():
+    """Q^2 Euler, data that vary along one axis only and have no momentum across it:
+    the fluxes of that momentum are the pressure, whose differences cancel exactly in
+    every mode but those of the faces' sums."""
+    for axis in (1, 2):  # the field without momentum: x, y
+        p, ctx = _pair(O.EULER, 2, O.BASIS_Q, 10, 9)
+        rng = np.random.default_rng(axis)
+        u = _state(p, rng, 0.05)
+        u[:, axis] = 0.0
+        for m, (a, b) in enumerate(p.modes()):
+            if (a if axis == 1 else b) > 0:
+                u[:, :, m] = 0.0
+        u[:] = u[:, :, :, :, :1] if axis == 1 else u[:, :, :, :1, :]
+        L = torch.zeros(p.shape, dtype=torch.float64, device="cuda")
+        ctx.cdg_rhs(torch.from_numpy(u).cuda(), 1e-3, L)
+        L = L.cpu().numpy()
+        for m, (a, b) in enumerate(p.modes()):
+            if (a if axis == 1 else b) == 0:
+                assert (L[:, axis, m] == 0.0).all(), (axis, m)
