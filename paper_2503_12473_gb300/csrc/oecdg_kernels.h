@@ -69,7 +69,6 @@ cudaError_t launch_persist1d(int sys, int bc, int k, const Geo& g, const Persist
 // 2D Q^k / P^k, k in {1, 2, 3}: every configuration outside the tiled Q^2 path
 long long partial_blocks_2k(const Geo& g, int k);
 int modes_2k(int k, int basis);
-int launches_stage2k(int sys, int basis, int rhs_only);  // kernels of one launch_stage2k
 cudaError_t launch_stage2k(int sys, int bc, int k, int basis, const Geo& g, int rhs_only, const double* uin,
                            const StageComb& cb, double* out, const double* dt, double* partials, cudaStream_t st);
 cudaError_t launch_oe2k(int sys, int bc, int k, int basis, const Geo& g, const double* uh, double* usig,
