@@ -113,3 +113,25 @@ def test_a_stage_is_the_combination_of_its_right_hand_side(k, basis, system, sid
     ctx.cdg_rk_stage(1, un, ul, out)
     ref = 0.75 * un + 0.25 * (ul + tau * L)
     assert float((out - ref).abs().max()) <= 1e-14 * float(ul.abs().max())
+
+
+@pytest.mark.parametrize("basis", [O.BASIS_Q, O.BASIS_P])
+def test_more_rows_than_a_grid_dimension_of_tiles(basis):
+    """131080 rows in tiles of 2 at k = 3: data of period 8 in y give the rows of the
+    8-row mesh, bit for bit (the cells are alike: h = 1 on both)."""
+    reps = 16385
+    p, small = _pair(O.ADVECTION, 3, basis, 3, 8, bx=3.0, by=8.0)
+    _, tall = _pair(O.ADVECTION, 3, basis, 3, 8 * reps, bx=3.0, by=8.0 * reps)
+    u = torch.from_numpy(_state(p, np.random.default_rng(1))).cuda()
+    v = u.repeat(1, 1, 1, reps, 1).contiguous()
+    a, b = torch.zeros_like(u), torch.zeros_like(v)
+    small.cdg_rhs(u, 1e-2, a)
+    tall.cdg_rhs(v, 1e-2, b)
+    assert torch.equal(b, a.repeat(1, 1, 1, reps, 1))
+    for ctx, x, out in ((small, u, a), (tall, v, b)):
+        ctx.cdg_set_dt(0.5e-2, 1e-2)
+        ctx.cdg_rk_stage(0, x, x, out)
+    assert torch.equal(b, a.repeat(1, 1, 1, reps, 1))
+    d, s = torch.zeros((2, 8 * reps, 3, 4), dtype=torch.float64, device="cuda"), torch.zeros((2, 1), dtype=torch.float64, device="cuda")
+    tall.cdg_oe_coefficients(v, d, s)
+    assert torch.equal(d, d[:, :8].repeat(1, reps, 1, 1)) and float(d.min()) > 0.0
