@@ -54,16 +54,15 @@ __global__ void k_sigma(const double* __restrict__ partials, long long nblk, int
 // over fields (Remark on systems); delta = 0 where sigma = 0.  Mode (a,b) then
 // decays by exp(-tau sum_{m <= min(a+b, 2)} delta^m), the average is kept.
 // Damping coefficients and the exact OE step of every cell (oe_warp2d).
-template <int SYS, int BC, bool WRITE_DELTA, bool ISO>
+template <int SYS, int BC, bool ISO>
 __global__ void __launch_bounds__(32 * STY, OECDG_OE_MINB) k_oe2d(Geo g, const double* __restrict__ uh,
                                                                   double* __restrict__ usig,
                                                                   const double* __restrict__ dt,
                                                                   const double* __restrict__ sigma,
-                                                                  double* __restrict__ delta_out,
                                                                   int* __restrict__ status) {
   __shared__ double isg[Fields<SYS>::F];
   oe_inv_sigma<Fields<SYS>::F>(sigma, blockIdx.x & 1, isg);
-  oe_warp2d<SYS, BC, WRITE_DELTA, 0, ISO, LD_NC>(g, uh, usig, dt, isg, delta_out, status, blockIdx.x & 1,
+  oe_warp2d<SYS, BC, 0, ISO, LD_NC>(g, uh, usig, dt, isg, status, blockIdx.x & 1,
                                                  (blockIdx.x >> 1) * SW_CELLS, blockIdx.y * STY + (threadIdx.x >> 5));
 }
 
@@ -233,27 +232,21 @@ cudaError_t launch_sigma(const double* partials, long long nblk, int F, const Si
 
 template <int SYS, int BC>
 static cudaError_t oe2d_t(const Geo& g, const double* uh, double* usig, const double* dt, const double* sigma,
-                          double* delta, int* status, cudaStream_t st) {
+                          int* status, cudaStream_t st) {
   // square cells: the isotropic variant of the OE body (same result up to rounding)
   const bool iso = g.hx == g.hy;
-  if (delta && iso)
-    k_oe2d<SYS, BC, true, true><<<stage_grid(g), 32 * STY, 0, st>>>(g, uh, usig, dt, sigma, delta, status);
-  else if (delta)
-    k_oe2d<SYS, BC, true, false><<<stage_grid(g), 32 * STY, 0, st>>>(g, uh, usig, dt, sigma, delta, status);
-  else if (iso)
-    k_oe2d<SYS, BC, false, true><<<stage_grid(g), 32 * STY, 0, st>>>(g, uh, usig, dt, sigma, delta, status);
-  else
-    k_oe2d<SYS, BC, false, false><<<stage_grid(g), 32 * STY, 0, st>>>(g, uh, usig, dt, sigma, delta, status);
+  if (iso) k_oe2d<SYS, BC, true><<<stage_grid(g), 32 * STY, 0, st>>>(g, uh, usig, dt, sigma, status);
+  else k_oe2d<SYS, BC, false><<<stage_grid(g), 32 * STY, 0, st>>>(g, uh, usig, dt, sigma, status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_oe2d(int sys, int bc, const Geo& g, const double* uh, double* usig, const double* dt,
-                        const double* sigma, double* delta, int* status, cudaStream_t st) {
+                        const double* sigma, int* status, cudaStream_t st) {
   auto go = [&](auto S) {
     constexpr int SYS = decltype(S)::value;
-    if (bc == BC_PERIODIC) return oe2d_t<SYS, BC_PERIODIC>(g, uh, usig, dt, sigma, delta, status, st);
-    if (bc == BC_TRANSMISSIVE) return oe2d_t<SYS, BC_TRANSMISSIVE>(g, uh, usig, dt, sigma, delta, status, st);
-    return oe2d_t<SYS, BC_GENERAL>(g, uh, usig, dt, sigma, delta, status, st);
+    if (bc == BC_PERIODIC) return oe2d_t<SYS, BC_PERIODIC>(g, uh, usig, dt, sigma, status, st);
+    if (bc == BC_TRANSMISSIVE) return oe2d_t<SYS, BC_TRANSMISSIVE>(g, uh, usig, dt, sigma, status, st);
+    return oe2d_t<SYS, BC_GENERAL>(g, uh, usig, dt, sigma, status, st);
   };
   if (sys == SYS_EULER) return go(std::integral_constant<int, SYS_EULER>{});
   return go(std::integral_constant<int, SYS_ADV>{});

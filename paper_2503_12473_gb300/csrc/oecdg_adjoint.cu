@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(AT, 4) k_oe_rec2d(Geo g, const double* __restr
                                                     int* __restrict__ status, double* __restrict__ rec) {
   __shared__ double isg[Fields<SYS>::F];
   oe_inv_sigma<Fields<SYS>::F>(sigma, blockIdx.z, isg);
-  oe_warp2d<SYS, BC_PERIODIC, false, 1, ISO, LD_NC>(g, uh, usig, dt, isg, nullptr, status, blockIdx.z,
+  oe_warp2d<SYS, BC_PERIODIC, 1, ISO, LD_NC>(g, uh, usig, dt, isg, status, blockIdx.z,
                                                    blockIdx.x * SW_CELLS, blockIdx.y * (AT / 32) + (threadIdx.x >> 5),
                                                    rec);
 }

@@ -286,11 +286,11 @@ static cudaError_t run_oe(cdg_ctx* ctx, const double* uh, double* usig, double* 
   if (e != cudaSuccess) return e;
   ctx->launches += 2;
   prof_mark(ctx, PROF_OE, 0);
-  if (!ctx->tiled2)
+  if (!ctx->tiled2 || delta)
     e = launch_oe2k(ctx->sys, ctx->bc, ctx->d.k, basis_of(ctx), ctx->g, uh, usig, ctx->dt, ctx->sigma, delta,
                     ctx->status, ctx->stream);
   else
-    e = launch_oe2d(ctx->sys, ctx->bc, ctx->g, uh, usig, ctx->dt, ctx->sigma, delta, ctx->status, ctx->stream);
+    e = launch_oe2d(ctx->sys, ctx->bc, ctx->g, uh, usig, ctx->dt, ctx->sigma, ctx->status, ctx->stream);
   prof_mark(ctx, PROF_OE, 1);
   return e;
 }

@@ -88,9 +88,9 @@ __device__ __forceinline__ void boe_tile(const BatchInst* __restrict__ I, int n,
   oe_inv_sigma<Fields<SYS>::F>(in.sigma, mesh, isg);
   // square cells: the isotropic variant, as the single-mesh launch chooses it
   if (in.g.hx == in.g.hy)
-    oe_warp2d<SYS, BC, false, 0, true, LD>(in.g, in.a, out, in.dt, isg, nullptr, status, mesh, i0, j);
+    oe_warp2d<SYS, BC, 0, true, LD>(in.g, in.a, out, in.dt, isg, status, mesh, i0, j);
   else
-    oe_warp2d<SYS, BC, false, 0, false, LD>(in.g, in.a, out, in.dt, isg, nullptr, status, mesh, i0, j);
+    oe_warp2d<SYS, BC, 0, false, LD>(in.g, in.a, out, in.dt, isg, status, mesh, i0, j);
 }
 
 template <int SYS, int BC, int R>

@@ -13,7 +13,7 @@ int wave_blocks_2d(const Geo& g);
 cudaError_t launch_stage2d(int sys, int bc, const Geo& g, int rhs_only, const double* uin, const double* un,
                            double* out, const double* dt, double ca, double cb, double* partials, cudaStream_t st);
 cudaError_t launch_oe2d(int sys, int bc, const Geo& g, const double* uh, double* usig, const double* dt,
-                        const double* sigma, double* delta, int* status, cudaStream_t st);
+                        const double* sigma, int* status, cudaStream_t st);
 cudaError_t launch_dt2d(int sys, const Geo& g, const double* u, double* partial, int nblk, double T_end, double* dt,
                         double* time, int* status, cudaStream_t st);
 cudaError_t launch_points2d(const Geo& g, double ax, double ay, double* xy, cudaStream_t st);
@@ -71,6 +71,7 @@ long long partial_blocks_2k(const Geo& g, int k);
 int modes_2k(int k, int basis);
 cudaError_t launch_stage2k(int sys, int bc, int k, int basis, const Geo& g, int rhs_only, const double* uin,
                            const StageComb& cb, double* out, const double* dt, double* partials, cudaStream_t st);
+// usig: the exact OE step; delta: the damping coefficients, in FP64 (either may be null)
 cudaError_t launch_oe2k(int sys, int bc, int k, int basis, const Geo& g, const double* uh, double* usig,
                         const double* dt, const double* sigma, double* delta, int* status, cudaStream_t st);
 cudaError_t launch_dt2k(int sys, int k, int basis, const Geo& g, const double* u, double* partial, int nblk,

@@ -135,3 +135,43 @@ def test_more_rows_than_a_grid_dimension_of_tiles(basis):
     d, s = torch.zeros((2, 8 * reps, 3, 4), dtype=torch.float64, device="cuda"), torch.zeros((2, 1), dtype=torch.float64, device="cuda")
     tall.cdg_oe_coefficients(v, d, s)
     assert torch.equal(d, d[:, :8].repeat(1, reps, 1, 1)) and float(d.min()) > 0.0
+
+
+def _delta(ctx, p, u):
+    d = torch.zeros((2, p.ny, p.nx, p.k + 1), dtype=torch.float64, device="cuda")
+    ctx.cdg_oe_coefficients(torch.from_numpy(u).cuda(), d, None)
+    return d.cpu().numpy()
+
+
+@pytest.mark.parametrize("along", [0, 1])
+@pytest.mark.parametrize("aspect", [10.0, 100.0, 1e4])
+@pytest.mark.parametrize("k,basis", KB)
+def test_coefficients_of_oblong_cells(k, basis, aspect, along):
+    """Data that vary along the longer side only: every cell's delta^m, whose derivatives
+    the m-th power of the aspect ratio scales down, to the rounding of some tens of terms
+    (a sum of norms, so nothing cancels behind the point values: 1e-12)."""
+    n, h = (8, 6), ((aspect, 1.0) if along == 0 else (1.0, aspect))
+    p, ctx = _pair(O.ADVECTION, k, basis, *n, bx=n[0] * h[0], by=n[1] * h[1])
+    u = np.random.default_rng(k).standard_normal(p.shape)
+    for m, ab in enumerate(p.modes()):
+        if ab[1 - along]:
+            u[:, :, m] = 0.0
+    u[:] = u[:, :, :, :1, :] if along == 0 else u[:, :, :, :, :1]
+    ref, _, _, st = O.oe_coefficients(p, u)
+    assert st == O.OK and ref.min() > 0.0
+    assert (np.abs(_delta(ctx, p, u) - ref) / ref).max() <= 1e-12
+
+
+@pytest.mark.parametrize("system", SYSTEMS)
+@pytest.mark.parametrize("k,basis", KB)
+def test_coefficients_far_below_the_variation(k, basis, system):
+    """Modes that fall off as 2^-8 per degree, as resolved data's: delta^k is taken from
+    the highest ones, exactly, whatever the size of the lower ones (1e-12 as above)."""
+    p, ctx = _pair(system, k, basis, 11, 6, by=0.5)
+    rng = np.random.default_rng(k)
+    u = _state(p, rng, 0.0)
+    for m, (a, b) in enumerate(p.modes()):
+        u[:, :, m] += 2.0 ** (-4 - 8 * (a + b)) * rng.uniform(0.5, 1.0, u[:, :, m].shape) * rng.choice([-1.0, 1.0], u[:, :, m].shape)
+    ref, _, _, st = O.oe_coefficients(p, u)
+    assert st == O.OK
+    assert (np.abs(_delta(ctx, p, u) - ref)[..., k] / ref[..., k]).max() <= 1e-12
