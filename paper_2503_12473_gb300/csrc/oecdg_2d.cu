@@ -54,7 +54,7 @@ __global__ void k_sigma(const double* __restrict__ partials, long long nblk, int
 // over fields (Remark on systems); delta = 0 where sigma = 0.  Mode (a,b) then
 // decays by exp(-tau sum_{m <= min(a+b, 2)} delta^m), the average is kept.
 // Damping coefficients and the exact OE step of every cell (oe_warp2d).
-template <int SYS, int BC, bool ISO>
+template <int SYS, int BC, int FORM>
 __global__ void __launch_bounds__(32 * STY, OECDG_OE_MINB) k_oe2d(Geo g, const double* __restrict__ uh,
                                                                   double* __restrict__ usig,
                                                                   const double* __restrict__ dt,
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(32 * STY, OECDG_OE_MINB) k_oe2d(Geo g, const d
                                                                   int* __restrict__ status) {
   __shared__ double isg[Fields<SYS>::F];
   oe_inv_sigma<Fields<SYS>::F>(sigma, blockIdx.x & 1, isg);
-  oe_warp2d<SYS, BC, 0, ISO, LD_NC>(g, uh, usig, dt, isg, status, blockIdx.x & 1,
+  oe_warp2d<SYS, BC, 0, FORM, LD_NC>(g, uh, usig, dt, isg, status, blockIdx.x & 1,
                                                  (blockIdx.x >> 1) * SW_CELLS, blockIdx.y * STY + (threadIdx.x >> 5));
 }
 
@@ -233,10 +233,10 @@ cudaError_t launch_sigma(const double* partials, long long nblk, int F, const Si
 template <int SYS, int BC>
 static cudaError_t oe2d_t(const Geo& g, const double* uh, double* usig, const double* dt, const double* sigma,
                           int* status, cudaStream_t st) {
-  // square cells: the isotropic variant of the OE body (same result up to rounding)
-  const bool iso = g.hx == g.hy;
-  if (iso) k_oe2d<SYS, BC, true><<<stage_grid(g), 32 * STY, 0, st>>>(g, uh, usig, dt, sigma, status);
-  else k_oe2d<SYS, BC, false><<<stage_grid(g), 32 * STY, 0, st>>>(g, uh, usig, dt, sigma, status);
+  const int form = oe_form(g);
+  if (form == OE_SQUARE) k_oe2d<SYS, BC, OE_SQUARE><<<stage_grid(g), 32 * STY, 0, st>>>(g, uh, usig, dt, sigma, status);
+  else if (form == OE_MILD) k_oe2d<SYS, BC, OE_MILD><<<stage_grid(g), 32 * STY, 0, st>>>(g, uh, usig, dt, sigma, status);
+  else k_oe2d<SYS, BC, OE_OBLONG><<<stage_grid(g), 32 * STY, 0, st>>>(g, uh, usig, dt, sigma, status);
   return cudaGetLastError();
 }
 

@@ -24,6 +24,8 @@
 #include <stdlib.h>
 
 #include "../../include/oecdg.h"
+#include <type_traits>
+
 #include "oecdg_2d_body.cuh"
 #include "oecdg_kernels.h"
 
@@ -544,15 +546,14 @@ __device__ __forceinline__ void beta_and_grad(const Geo& g, const double* w, dou
 
 // Forward OE step that also records (delta^m, field of the max, its face
 // sums) per cell for the adjoint.
-template <int SYS, bool ISO>
+template <int SYS, int FORM>
 __global__ void __launch_bounds__(AT, 4) k_oe_rec2d(Geo g, const double* __restrict__ uh, double* __restrict__ usig,
                                                     const double* __restrict__ dt, const double* __restrict__ sigma,
                                                     int* __restrict__ status, double* __restrict__ rec) {
   __shared__ double isg[Fields<SYS>::F];
   oe_inv_sigma<Fields<SYS>::F>(sigma, blockIdx.z, isg);
-  oe_warp2d<SYS, BC_PERIODIC, 1, ISO, LD_NC>(g, uh, usig, dt, isg, status, blockIdx.z,
-                                                   blockIdx.x * SW_CELLS, blockIdx.y * (AT / 32) + (threadIdx.x >> 5),
-                                                   rec);
+  oe_warp2d<SYS, BC_PERIODIC, 1, FORM, LD_NC>(g, uh, usig, dt, isg, status, blockIdx.z, blockIdx.x * SW_CELLS,
+                                              blockIdx.y * (AT / 32) + (threadIdx.x >> 5), rec);
 }
 
 // Reverse of one derivative order M of the face sums of one field: given the
@@ -1127,10 +1128,14 @@ static cudaError_t adj_forward(cdg_ctx* c, const double* un, double* const* H, d
     if (oe) {
       if ((e = launch_sigma(c->partials, c->nblk, F, plain_norm(g.plane), c->sigma, c->avg, st)) != cudaSuccess) return e;
       const dim3 grid((g.nx + SW_CELLS - 1) / SW_CELLS, (g.ny + AT / 32 - 1) / (AT / 32), 2);
-      // the variant the forward step uses (square cells: isotropic), so the
-      // recorded states equal cdg_step's
-      if (g.hx == g.hy) k_oe_rec2d<SYS, true><<<grid, AT, 0, st>>>(g, H[l], dst, dt, c->sigma, c->status, R[l]);
-      else k_oe_rec2d<SYS, false><<<grid, AT, 0, st>>>(g, H[l], dst, dt, c->sigma, c->status, R[l]);
+      // the form the forward step uses, so the recorded states equal cdg_step's
+      const int form = oe_form(g);
+      auto rec = [&](auto Fm) {
+        k_oe_rec2d<SYS, decltype(Fm)::value><<<grid, AT, 0, st>>>(g, H[l], dst, dt, c->sigma, c->status, R[l]);
+      };
+      if (form == OE_SQUARE) rec(std::integral_constant<int, OE_SQUARE>{});
+      else if (form == OE_MILD) rec(std::integral_constant<int, OE_MILD>{});
+      else rec(std::integral_constant<int, OE_OBLONG>{});
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     } else if ((e = cudaMemcpyAsync(dst, H[l], c->numel * sizeof(double), cudaMemcpyDeviceToDevice, st)) !=
                cudaSuccess) {

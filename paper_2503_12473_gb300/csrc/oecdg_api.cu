@@ -272,7 +272,7 @@ static StageComb comb2(const double* u0, double c0, const double* u1, double c1,
 }
 
 // sigma from the partials of the last stage kernel, then the OE kernel (1D:
-// both in one launch)
+// both in one launch); with delta the damping coefficients instead (usig is null)
 static cudaError_t run_oe(cdg_ctx* ctx, const double* uh, double* usig, double* delta) {
   if (ctx->d.dim == 1) {
     ctx->launches += 1;
@@ -286,9 +286,12 @@ static cudaError_t run_oe(cdg_ctx* ctx, const double* uh, double* usig, double* 
   if (e != cudaSuccess) return e;
   ctx->launches += 2;
   prof_mark(ctx, PROF_OE, 0);
-  if (!ctx->tiled2 || delta)
-    e = launch_oe2k(ctx->sys, ctx->bc, ctx->d.k, basis_of(ctx), ctx->g, uh, usig, ctx->dt, ctx->sigma, delta,
-                    ctx->status, ctx->stream);
+  if (delta)
+    e = launch_delta2k(ctx->sys, ctx->bc, ctx->d.k, basis_of(ctx), ctx->g, uh, delta, ctx->dt, ctx->sigma,
+                       ctx->status, ctx->stream);
+  else if (!ctx->tiled2)
+    e = launch_oe2k(ctx->sys, ctx->bc, ctx->d.k, basis_of(ctx), ctx->g, uh, usig, ctx->dt, ctx->sigma, ctx->status,
+                    ctx->stream);
   else
     e = launch_oe2d(ctx->sys, ctx->bc, ctx->g, uh, usig, ctx->dt, ctx->sigma, ctx->status, ctx->stream);
   prof_mark(ctx, PROF_OE, 1);

@@ -86,11 +86,10 @@ __device__ __forceinline__ void boe_tile(const BatchInst* __restrict__ I, int n,
   const int i0 = (t % in.tx) * SW_CELLS, j = (t / in.tx) * R + (threadIdx.x >> 5);
   double* out = last ? in.u : in.b;
   oe_inv_sigma<Fields<SYS>::F>(in.sigma, mesh, isg);
-  // square cells: the isotropic variant, as the single-mesh launch chooses it
-  if (in.g.hx == in.g.hy)
-    oe_warp2d<SYS, BC, 0, true, LD>(in.g, in.a, out, in.dt, isg, status, mesh, i0, j);
-  else
-    oe_warp2d<SYS, BC, 0, false, LD>(in.g, in.a, out, in.dt, isg, status, mesh, i0, j);
+  const int form = oe_form(in.g);  // as the single-mesh launch
+  if (form == OE_SQUARE) oe_warp2d<SYS, BC, 0, OE_SQUARE, LD>(in.g, in.a, out, in.dt, isg, status, mesh, i0, j);
+  else if (form == OE_MILD) oe_warp2d<SYS, BC, 0, OE_MILD, LD>(in.g, in.a, out, in.dt, isg, status, mesh, i0, j);
+  else oe_warp2d<SYS, BC, 0, OE_OBLONG, LD>(in.g, in.a, out, in.dt, isg, status, mesh, i0, j);
 }
 
 template <int SYS, int BC, int R>

@@ -5,6 +5,7 @@
 
 #include <cuda_runtime.h>
 #include <limits.h>
+#include <math.h>
 #include <stdint.h>
 
 namespace oecdg {
@@ -117,7 +118,8 @@ __device__ __forceinline__ double sqrt_pos(double x) {
 //             5 hy/24;
 //   oec:      of the Q^2 OE kernel, x- then y-faces: 32/9 (the unit of its
 //             integer sums) x 1/(12 h), 1/4, 5 h/24 x (2/min(hx, hy))^m;
-//   rho_x, rho_y: min(hx, hy)/hx and min(hx, hy)/hy times 2^62, below 2^62.
+//   rho, rho_x: (h_min / h_max)^al = rho[al - 1] 2^(-62 - rho_x[al - 1]), al = 1..3,
+//             rho[.] in [2^61, 2^62).
 struct Geo {
   int nx, ny;
   long long plane;
@@ -129,7 +131,8 @@ struct Geo {
   int bcs[4];
   double i1x, i1y, i2x, i2y, i12x, i12y, h24x5, h24y5;
   double oec[6];
-  long long rho_x, rho_y;
+  long long rho[3];
+  int rho_x[3];
 };
 
 // The cell-size constants of Geo, from hx and hy (the same expressions the
@@ -149,9 +152,15 @@ inline void finish_geo(Geo& g) {
   g.oec[2] = c * g.h24x5 * (i2 * i2);
   g.oec[3] = c * g.i12y;
   g.oec[5] = c * g.h24y5 * (i2 * i2);
-  const long long one = 0x3fffffffffffffffLL;  // 2^62 - 1
-  g.rho_x = g.i2x < i2 ? (long long)(g.i2x / i2 * 0x1p62) : one;
-  g.rho_y = g.i2y < i2 ? (long long)(g.i2y / i2 * 0x1p62) : one;
+  const double r = (g.i2x < g.i2y ? g.i2x : g.i2y) / i2;
+  double p = 1.0;
+  for (int al = 0; al < 3; ++al) {
+    p *= r;
+    int e;
+    const double m = frexp(p, &e);
+    g.rho[al] = e > 0 ? 0x3fffffffffffffffLL : (long long)(m * 0x1p62);  // e > 0: rho = 1
+    g.rho_x[al] = e > 0 ? 0 : -e;
+  }
 }
 
 // 1/sigma of the F fields of `mesh` into shared isg[F] by the block's first

@@ -71,9 +71,13 @@ long long partial_blocks_2k(const Geo& g, int k);
 int modes_2k(int k, int basis);
 cudaError_t launch_stage2k(int sys, int bc, int k, int basis, const Geo& g, int rhs_only, const double* uin,
                            const StageComb& cb, double* out, const double* dt, double* partials, cudaStream_t st);
-// usig: the exact OE step; delta: the damping coefficients, in FP64 (either may be null)
 cudaError_t launch_oe2k(int sys, int bc, int k, int basis, const Geo& g, const double* uh, double* usig,
-                        const double* dt, const double* sigma, double* delta, int* status, cudaStream_t st);
+                        const double* dt, const double* sigma, int* status, cudaStream_t st);
+cudaError_t launch_oe2k_oblong(int sys, int bc, int k, int basis, const Geo& g, const double* uh, double* usig,
+                               const double* dt, const double* sigma, int* status, cudaStream_t st);
+// delta^0..delta^k of every cell, in FP64 (every 2D space, Q^2 included)
+cudaError_t launch_delta2k(int sys, int bc, int k, int basis, const Geo& g, const double* uh, double* delta,
+                           const double* dt, const double* sigma, int* status, cudaStream_t st);
 cudaError_t launch_dt2k(int sys, int k, int basis, const Geo& g, const double* u, double* partial, int nblk,
                         double T_end, double* dt, double* time, int* status, cudaStream_t st);
 cudaError_t launch_points2k(int k, const Geo& g, double ax, double ay, double bx, double by, double* xy,

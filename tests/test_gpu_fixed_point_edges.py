@@ -175,3 +175,28 @@ def test_coefficients_far_below_the_variation(k, basis, system):
     ref, _, _, st = O.oe_coefficients(p, u)
     assert st == O.OK
     assert (np.abs(_delta(ctx, p, u) - ref)[..., k] / ref[..., k]).max() <= 1e-12
+
+
+@pytest.mark.parametrize("along", [0, 1])
+@pytest.mark.parametrize("aspect", [8.0, 64.0, 1e4])
+@pytest.mark.parametrize("k,basis", KB)
+def test_damping_of_oblong_cells(k, basis, aspect, along):
+    """Averages that vary along the longer side, modes of degree 1 and more along the
+    shorter one by 2^-s smaller (s = 0..40: from complete decay to none), h_min = 1, tau =
+    0.1: a decay's argument rounds some 50 times, 0.37 x 50 x 2^-53 of the largest mode."""
+    n, h = (8, 6), ((aspect, 1.0) if along == 0 else (1.0, aspect))
+    p, ctx = _pair(O.ADVECTION, k, basis, *n, bx=n[0] * h[0], by=n[1] * h[1])
+    ctx.cdg_set_dt(0.1, 0.1)
+    for s in range(0, 44, 4):
+        rng = np.random.default_rng(s)
+        u = rng.standard_normal(p.shape)
+        u[:, :, 0] = u[:, :, 0, :1, :] if along == 0 else u[:, :, 0, :, :1]
+        for m, ab in enumerate(p.modes()):
+            if ab[1 - along]:
+                u[:, :, m] *= 2.0 ** -s
+        ug = torch.from_numpy(u).cuda()
+        out = torch.zeros_like(ug)
+        ctx.cdg_oe_damp(ug, out)
+        ref, st = O.oe(p, u, 0.1)
+        assert st == O.OK
+        assert np.abs(out.cpu().numpy() - ref).max() <= 2e-15 * np.abs(u).max(), s
