@@ -131,7 +131,12 @@ cdg_status cdg_project_ic(cdg_ctx* ctx, const double* d_vals, double* d_u);
 
 /* Semi-discrete right-hand side of the CDG method, Eq. (equcdg) (1D Eq.
  * (eq:1D_H), 2D Eq. (eq:2D_H)): d_L = M^{-1} H(u, .) on both meshes, with the
- * dissipation coefficient 1/tau_max.  d_L must not alias d_u. */
+ * dissipation coefficient 1/tau_max.  d_L must not alias d_u.
+ * 2D kernels (stages, steps and batches too) form the linear sums of a cell in 64-bit
+ * fixed point relative to its largest coefficient of the field.  The range is that of a
+ * double, but for a cell's field that is below 2^-959 throughout: it is held to 2^-1019
+ * absolute, and results below 2^-1022 are 0.  A value that is not finite makes the
+ * results that it enters NaN (or, from its cell's own coefficients alone, infinite). */
 cdg_status cdg_rhs(cdg_ctx* ctx, const double* d_u, double tau_max, double* d_L);
 
 /* Time step of Section 4 (2D: tau_max = C_CFL / (beta_x/h_x + beta_y/h_y);

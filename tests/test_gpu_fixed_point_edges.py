@@ -200,3 +200,44 @@ def test_damping_of_oblong_cells(k, basis, aspect, along):
         ref, st = O.oe(p, u, 0.1)
         assert st == O.OK
         assert np.abs(out.cpu().numpy() - ref).max() <= 2e-15 * np.abs(u).max(), s
+
+
+@pytest.mark.parametrize("power", [1018, -930])
+@pytest.mark.parametrize("k,basis", KB)
+def test_linear_results_scale_with_the_data(k, basis, power):
+    """Advection of data times a power of two, up to the last ones whose sums are finite:
+    right-hand side, stage and damping are the unscaled ones times it, bit for bit (2 x 2
+    cells, so that the sum of the averages is finite too)."""
+    p, ctx = _pair(O.ADVECTION, k, basis, 2, 2)
+    u = torch.from_numpy(0.5 * _state(p, np.random.default_rng(k), 0.05)).cuda()
+    tau, tm = 2.0 ** -9, 2.0 ** -8
+    ctx.cdg_set_dt(tau, tm)
+    s, got = 2.0 ** power, []
+    for x in (u, u * s):
+        L, stage, damped = torch.zeros_like(u), torch.zeros_like(u), torch.zeros_like(u)
+        ctx.cdg_rhs(x, 1.0, L)
+        ctx.cdg_rk_stage(0, x, x, stage)
+        ctx.cdg_oe_damp(x, damped)
+        got.append((L, stage, damped))
+    for a, b in zip(*got):
+        assert torch.isfinite(b).all() and torch.equal(a * s, b)
+
+
+@pytest.mark.parametrize("system", SYSTEMS)
+@pytest.mark.parametrize("k,basis", KB)
+def test_infinities_and_nans_give_nan(k, basis, system):
+    """One value that is not finite makes the right-hand side NaN in the cells that
+    overlap it, and no other."""
+    for bad in (float("inf"), float("-inf"), float("nan")):
+        p, ctx = _pair(system, k, basis, 12, 7)
+        u = _state(p, np.random.default_rng(k))
+        u[0, 0, 0, 3, 5] = bad
+        L = torch.zeros(p.shape, dtype=torch.float64, device="cuda")
+        ctx.cdg_rhs(torch.from_numpy(u).cuda(), 1e-3, L)
+        L = L.cpu().numpy()
+        finite = np.isfinite(L).all(axis=(1, 2))
+        near = np.zeros(finite.shape, bool)
+        near[1, 2:4, 4:6] = True  # dual cells over primal (5, 3)
+        near[0, 3, 5] = True  # its own -u / tau term
+        assert (finite == ~near).all()
+        assert np.isnan(L[1, 0, 0, 2:4, 4:6]).all()
