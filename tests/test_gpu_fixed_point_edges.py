@@ -241,3 +241,20 @@ def test_infinities_and_nans_give_nan(k, basis, system):
         near[0, 3, 5] = True  # its own -u / tau term
         assert (finite == ~near).all()
         assert np.isnan(L[1, 0, 0, 2:4, 4:6]).all()
+
+
+@pytest.mark.parametrize("system", SYSTEMS)
+@pytest.mark.parametrize("k,basis", KB)
+def test_a_nan_mode_leaves_sigma_to_the_other_cells(k, basis, system):
+    """One cell's highest mode is NaN beside the cells that hold the extrema of their
+    fields: that mesh's sigma is the one without the cell's variation."""
+    p, ctx = _pair(system, k, basis, 12, 7)
+    u = _state(p, np.random.default_rng(k))
+    u[0, :, 0, 0, 0] += 0.3  # the extremum, in the same tile
+    u[0, :, 1:, 0, 3] = 0.0
+    v = u.copy()
+    v[0, :, -1, 0, 3] = np.nan
+    s, t = (torch.zeros((2, p.nfields), dtype=torch.float64, device="cuda") for _ in range(2))
+    ctx.cdg_oe_coefficients(torch.from_numpy(u).cuda(), None, s)
+    ctx.cdg_oe_coefficients(torch.from_numpy(v).cuda(), None, t)
+    assert float(s.min()) > 0.0 and torch.equal(s[0], t[0])
