@@ -389,7 +389,7 @@ __global__ void k_acc_partials(const double* __restrict__ part, long long n, dou
 
 // (value, index) reductions on the integer pipes: the value as its
 // order-preserving key; the larger (smaller) value wins, ties go to the smaller
-// index.  NaN never wins.
+// index.  NaN (max_key, min_key: beyond both infinities) never wins over NO_MAX, NO_MIN.
 struct Extreme {
   long long key, at;
 };
@@ -402,6 +402,7 @@ __device__ __forceinline__ void argmin_merge(Extreme& a, long long key, long lon
 // -0 and +0 are one value: the key of +0 for both
 __device__ __forceinline__ double plus_zero(double v) { return __double_as_longlong(v) == LLONG_MIN ? 0.0 : v; }
 constexpr long long NO_POINT = LLONG_MAX;
+constexpr Extreme NO_MAX = {-0x7ff0000000000001LL, NO_POINT}, NO_MIN = {0x7ff0000000000000LL, NO_POINT};  // -inf, inf
 
 __device__ __forceinline__ void warp_argmax(Extreme& a) {
   const unsigned full = 0xffffffffu;
@@ -438,7 +439,7 @@ __global__ void __launch_bounds__(256) k_sigma_stats2d(Geo g, const double* __re
 #pragma unroll
     for (int m = 0; m < 9; ++m) v[m] = us[(f * 9 + m) * g.plane];
     double s = active ? v[0] : 0.0;
-    Extreme mx = {LLONG_MIN, NO_POINT}, mn = {LLONG_MAX, NO_POINT};
+    Extreme mx = NO_MAX, mn = NO_MIN;
     if (active) {
 #pragma unroll
       for (int qy = 0; qy < 3; ++qy) {
@@ -465,8 +466,8 @@ __global__ void __launch_bounds__(256) k_sigma_stats2d(Geo g, const double* __re
     __syncthreads();
     if (warp == 0) {
       s = lane < nw ? sh[lane] : 0.0;
-      mx = lane < nw ? smx[lane] : Extreme{LLONG_MIN, NO_POINT};
-      mn = lane < nw ? smn[lane] : Extreme{LLONG_MAX, NO_POINT};
+      mx = lane < nw ? smx[lane] : NO_MAX;
+      mn = lane < nw ? smn[lane] : NO_MIN;
       warp_stats(s, mx, mn);
       if (lane == 0) {
         double* p = part + ((mesh * nblk + blockIdx.x) * F + f) * 5;
@@ -485,7 +486,7 @@ __global__ void k_sigma_stats_final(const double* __restrict__ part, long long n
                                     double* __restrict__ stats) {
   const int f = blockIdx.x, mesh = blockIdx.y;
   double s = 0.0;
-  Extreme mx = {LLONG_MIN, NO_POINT}, mn = {LLONG_MAX, NO_POINT};
+  Extreme mx = NO_MAX, mn = NO_MIN;
   for (long long b = threadIdx.x; b < nblk; b += 32) {
     const double* p = part + ((mesh * nblk + b) * F + f) * 5;
     s += p[0];
