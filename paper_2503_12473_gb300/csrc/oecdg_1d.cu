@@ -278,7 +278,7 @@ template <int SYS, int BC, int K, int MODE, int LD = LD_NC>
 __device__ __forceinline__ void stage_cell1d_2l(const Geo& g, const double* __restrict__ uin, const StageComb& cb,
                                                 double* __restrict__ out, const double* __restrict__ dt,
                                                 double* __restrict__ pblk, int mesh, int i, int sx) {
-  constexpr int F = Fields1<SYS>::F, M = K + 1, N = K + 1;
+  constexpr int F = Fields1<SYS>::F, M = K + 1;
   const unsigned full = 0xffffffffu;
   const bool active = i < cells_x(g, mesh);
   const int ic = active ? i : 0;

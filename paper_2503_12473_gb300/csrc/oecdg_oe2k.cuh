@@ -81,9 +81,7 @@ __global__ void __launch_bounds__(NTK, Modes2<K, B>::M > 10 ? 2 : (K > 2 ? 3 : 4
           t += __shfl_xor_sync(full, t, 16);
           if (f == fq) T[n][m] = __double_as_longlong(t);
         }
-      continue;
-    }
-    if constexpr (FORM == OEK_OBLONG) {
+    } else if constexpr (FORM == OEK_OBLONG) {
       const bool swap = g.hx < g.hy;
       fx s[2][K + 1];
       int E[K + 1];
@@ -99,47 +97,47 @@ __global__ void __launch_bounds__(NTK, Modes2<K, B>::M > 10 ? 2 : (K > 2 ? 3 : 4
         }
         if (f == fq) ev[m] = E[m];
       }
-      continue;
-    }
-    double k[M], o[M];
+    } else {
+      double k[M], o[M];
 #pragma unroll
-    for (int m = 0; m < M; ++m) {
-      k[m] = __ldg(us + (long long)(f * M + m) * P);
-      o[m] = __ldg(uo + (long long)(f * M + m) * P);
-    }
-    if (neg) o[0] = -o[0];
-    o[0] -= k[0];  // the means' difference; K's own mean counts as 0
-    unsigned mag = fx_mag(o[0]);
-#pragma unroll
-    for (int m = 1; m < M; ++m) mag = max(mag, max(fx_mag(k[m]), fx_mag(o[m])));
-    int ex = fx_exp(mag);
-    ex = max(ex, __shfl_xor_sync(full, ex, 8));
-    ex = max(ex, __shfl_xor_sync(full, ex, 16));
-    fx kc[M], oc[M];
-    kc[0] = 0;
-    oc[0] = to_fx<OEK_FX>(o[0], ex);
-#pragma unroll
-    for (int m = 1; m < M; ++m) {
-      const unsigned fk = (MD::a(m) & 1 ? (unsigned)sx : 0u) ^ (MD::b(m) & 1 ? (unsigned)sy : 0u);
-      const unsigned fo = fk ^ (MD::a(m) & 1 ? (unsigned)mx : 0u) ^ (MD::b(m) & 1 ? (unsigned)my : 0u) ^ (unsigned)neg;
-      kc[m] = to_fx<OEK_FX>(k[m], ex, fk << 31);
-      oc[m] = to_fx<OEK_FX>(o[m], ex, fo << 31);
-    }
-    fx s[2][K + 1];
-    oek_half_face<K, B, 0>(kc, oc, s[0]);
-    oek_half_face<K, B, 1>(kc, oc, s[1]);
-#pragma unroll
-    for (int n = 0; n < 2; ++n)
-#pragma unroll
-      for (int m = 0; m <= K; ++m) {
-        fx t = s[n][m];
-        t += shfl_xor_fx(t, 8);
-        t += shfl_xor_fx(t, 16);
-        if (f == fq) T[n][m] = t;
+      for (int m = 0; m < M; ++m) {
+        k[m] = __ldg(us + (long long)(f * M + m) * P);
+        o[m] = __ldg(uo + (long long)(f * M + m) * P);
       }
+      if (neg) o[0] = -o[0];
+      o[0] -= k[0];  // the means' difference; K's own mean counts as 0
+      unsigned mag = fx_mag(o[0]);
 #pragma unroll
-    for (int m = 0; m <= K; ++m)
-      if (f == fq) ev[m] = ex;
+      for (int m = 1; m < M; ++m) mag = max(mag, max(fx_mag(k[m]), fx_mag(o[m])));
+      int ex = fx_exp(mag);
+      ex = max(ex, __shfl_xor_sync(full, ex, 8));
+      ex = max(ex, __shfl_xor_sync(full, ex, 16));
+      fx kc[M], oc[M];
+      kc[0] = 0;
+      oc[0] = to_fx<OEK_FX>(o[0], ex);
+#pragma unroll
+      for (int m = 1; m < M; ++m) {
+        const unsigned fk = (MD::a(m) & 1 ? (unsigned)sx : 0u) ^ (MD::b(m) & 1 ? (unsigned)sy : 0u);
+        const unsigned fo = fk ^ (MD::a(m) & 1 ? (unsigned)mx : 0u) ^ (MD::b(m) & 1 ? (unsigned)my : 0u) ^ (unsigned)neg;
+        kc[m] = to_fx<OEK_FX>(k[m], ex, fk << 31);
+        oc[m] = to_fx<OEK_FX>(o[m], ex, fo << 31);
+      }
+      fx s[2][K + 1];
+      oek_half_face<K, B, 0>(kc, oc, s[0]);
+      oek_half_face<K, B, 1>(kc, oc, s[1]);
+#pragma unroll
+      for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int m = 0; m <= K; ++m) {
+          fx t = s[n][m];
+          t += shfl_xor_fx(t, 8);
+          t += shfl_xor_fx(t, 16);
+          if (f == fq) T[n][m] = t;
+        }
+#pragma unroll
+      for (int m = 0; m <= K; ++m)
+        if (f == fq) ev[m] = ex;
+    }
   }
 
   // wave speeds at the cell average, delta^m of field fq, the maximum over the fields

@@ -42,14 +42,14 @@ __device__ __forceinline__ void oek_nodes(const fx (&p)[4], fx (&v)[N]) {
 // 1/8 of the rule's sum (N = 3: of 9/4 of it)
 template <int N>
 __device__ __forceinline__ fx oek_rule(const fx (&v)[N]) {
-  fx w;
-  if constexpr (N == 2) w = v[0] + v[1];
-  else if constexpr (N == 3) {
+  if constexpr (N == 2) {
+    return (v[0] + v[1] + 4) >> 3;
+  } else if constexpr (N == 3) {
     const fx h = (v[0] + v[2]) >> 1;
     return (h + ((h + 2) >> 2) + v[1] + 2) >> 2;
+  } else {
+    return ((fx_mul(v[0] + v[1], FXN4_W_IN_2) << 1) + fx_mul(v[2] + v[3], FXN4_W_OUT) + 4) >> 3;
   }
-  else w = (fx_mul(v[0] + v[1], FXN4_W_IN_2) << 1) + fx_mul(v[2] + v[3], FXN4_W_OUT);
-  return (w + 4) >> 3;
 }
 constexpr double oek_rule_unit(int N) { return N == 3 ? 32.0 / 9.0 : 8.0; }
 
