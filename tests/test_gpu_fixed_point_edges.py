@@ -258,3 +258,50 @@ def test_a_nan_mode_leaves_sigma_to_the_other_cells(k, basis, system):
     ctx.cdg_oe_coefficients(torch.from_numpy(u).cuda(), None, s)
     ctx.cdg_oe_coefficients(torch.from_numpy(v).cuda(), None, t)
     assert float(s.min()) > 0.0 and torch.equal(s[0], t[0])
+
+
+@pytest.mark.parametrize("gamma", [1.0 + 2.0 ** -10, 1.4, 3.0])
+@pytest.mark.parametrize("low", [0.5, 2.0 ** -4, 2.0 ** -6, 2.0 ** -7, 2.0 ** -10, -(2.0 ** -10), -0.25])
+def test_fluxes_at_densities_close_to_zero(low, gamma):
+    """Q^2 Euler: cells whose density falls to `low` at one Gauss point, at every place of an
+    8-cell warp and in the ragged tile.  The largest flux of such a quarter is far below the
+    product of its factors' exponents, so its warp takes the fluxes in FP64; on either
+    side of that line.  A density rounds at about 2^-53 x 8 there and its flux by twice
+    the quotient: 2e-15 / |low|, and some tens of roundings in the sums: 1e-13 / min(1,
+    |low|) of a field's largest right-hand side."""
+    p, ctx = _pair(O.EULER, 2, O.BASIS_Q, 11, 6, bx=11 / 8, by=6 / 8, gamma=gamma)
+    u = _state(p, np.random.default_rng(3))
+    x = 0.5 + 0.5 * 0.6 ** 0.5  # the quarter's outer Gauss point in the overlapping cell
+    for mesh in range(2):
+        for n in range(8):
+            cell = (3 * n) % p.ny, n if mesh == 0 else n + 3
+            u[(mesh, 0, slice(1, None)) + cell] = 0.0
+            u[(mesh, 0, 0) + cell] = 1.0
+            u[(mesh, 0, 1) + cell] = (-1.0) ** n * (1.0 - low) / x
+    L = torch.zeros(p.shape, dtype=torch.float64, device="cuda")
+    ctx.cdg_rhs(torch.from_numpy(u).cuda(), 1 / 64, L)
+    ref = O.rhs(p, u, 1 / 64)
+    err = np.abs(L.cpu().numpy() - ref).max(axis=(0, 2, 3, 4)) / np.abs(ref).max(axis=(0, 2, 3, 4))
+    assert err.max() <= 1e-13 / min(1.0, abs(low)), err
+
+
+@pytest.mark.parametrize("gamma", [1.0 + 2.0 ** -10, 1.4, 3.0])
+@pytest.mark.parametrize("speed", [0.0, 1e-6, 1e3])
+def test_cells_at_rest_and_cold_fast_flow(speed, gamma):
+    """Q^2 Euler at Mach numbers from 0 to some thousands: the energy and momentum fluxes
+    to 1e-13 of the largest of their equations' terms (flux over h, the state over tau)."""
+    p, ctx = _pair(O.EULER, 2, O.BASIS_Q, 11, 6, bx=11 / 8, by=6 / 8, gamma=gamma)
+    rng = np.random.default_rng(5)
+    u = _state(p, rng)
+    u[:, 1:3] = 0.0
+    if speed:
+        u[:, 1, 0] = speed * (1.0 + 0.01 * rng.standard_normal(u[:, 1, 0].shape))
+        u[:, 2, 1:] = 1e-3 * speed * rng.standard_normal(u[:, 2, 1:].shape)
+        u[:, 3, 0] += 0.6 * speed ** 2
+    L = torch.zeros(p.shape, dtype=torch.float64, device="cuda")
+    ctx.cdg_rhs(torch.from_numpy(u).cuda(), 1 / 64, L)
+    ref = O.rhs(p, u, 1 / 64)
+    top = np.abs(u[:, 3]).max()
+    scale = np.array([1.0 + speed, top, top, top * (1.0 + speed)]) * 64 * 9
+    err = np.abs(L.cpu().numpy() - ref).max(axis=(0, 2, 3, 4)) / scale
+    assert err.max() <= 1e-13, err
