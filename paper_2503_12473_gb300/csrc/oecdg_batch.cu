@@ -702,14 +702,16 @@ cdg_status cdg_batch_rows(const cdg_batch* B, int* rows) {
   return CDG_OK;
 }
 
-// signature of a batch for the autotune cache: sizes, boundary and count
+// Signature of a batch for the autotune cache: the kernels' generation, sizes, boundary and
+// count.  The generation (fx1: fixed point, tiles 8 cells wide) is raised with every change
+// of what a choice of rows and grid stands for, so that a file tuned before is not used.
 static void batch_signature(const cdg_batch* B, char* sig, size_t len) {
   unsigned long long h = 1469598103934665603ULL;
   for (int q = 0; q < B->n; ++q) {
     h = (h ^ (unsigned long long)B->h_inst[q].g.nx) * 1099511628211ULL;
     h = (h ^ (unsigned long long)B->h_inst[q].g.ny) * 1099511628211ULL;
   }
-  snprintf(sig, len, "euler_q2_bc%d_n%d_%016llx", B->bc, B->n, h);
+  snprintf(sig, len, "euler_q2_fx1_bc%d_n%d_%016llx", B->bc, B->n, h);
 }
 
 static int cache_lookup(const char* path, const char* sig) {

@@ -1,4 +1,6 @@
 """The integer-pipe kernels of the 2D path at the edges of what they take."""
+import json
+
 import numpy as np
 import pytest
 
@@ -305,3 +307,26 @@ def test_cells_at_rest_and_cold_fast_flow(speed, gamma):
     scale = np.array([1.0 + speed, top, top, top * (1.0 + speed)]) * 64 * 9
     err = np.abs(L.cpu().numpy() - ref).max(axis=(0, 2, 3, 4)) / scale
     assert err.max() <= 1e-13, err
+
+
+def test_a_tuning_file_of_other_kernels_is_not_used(tmp_path):
+    """An entry without the kernels' generation (as the FP64 kernels wrote it) is kept in
+    the file, and the batch is tuned anew."""
+    from paper_2503_12473_gb300 import oecdg as G
+    descs = [G.MeshDesc(dim=2, nx=nx, ny=ny, system=G.EULER, bc=G.PERIODIC, cfl=0.1) for nx, ny in ((8, 12), (20, 9))]
+    h = 1469598103934665603
+    for d in descs:
+        for n in (d.nx, d.ny):
+            h = (h ^ n) * 1099511628211 % 2 ** 64
+    old = {f"euler_q2_bc0_n2_{h:016x}": 801}
+    path = tmp_path / "tune.json"
+    path.write_text(json.dumps(old))
+    us = []
+    for d in descs:
+        p = O.Problem(dim=2, nx=d.nx, ny=d.ny, k=2, system=O.EULER, bc=O.PERIODIC)
+        us.append(torch.from_numpy(_state(p, np.random.default_rng(d.nx))).cuda())
+    b = G.Batch(descs)
+    rows = b.cdg_batch_autotune(us, str(path))
+    new = json.loads(path.read_text())
+    assert len(new) == 2 and new.pop(next(iter(old))) == 801
+    assert list(new.values()) == [100 * rows + b.cdg_batch_grid()[0]]
