@@ -76,8 +76,10 @@ __global__ void __launch_bounds__(32 * R, R == 8 ? 1 : 12 / R) k_bstage(const Ba
   bstage_tile<SYS, BC, R, LD_NC>(I, n, blockIdx.x, l, ca, cb, smem);
 }
 
-// OE block `blk` of the batch: the damping coefficients and the OE step of its tile
-template <int SYS, int BC, int R, int LD>
+// OE block `blk` of the batch: the damping coefficients and the OE step of its tile.
+// SQUARE: every instance has square cells (with the other forms beside it the kernel of
+// 256 such meshes spills registers: a step of 11 launches 446.0 ms, against 443.6)
+template <int SYS, int BC, int R, int LD, bool SQUARE>
 __device__ __forceinline__ void boe_tile(const BatchInst* __restrict__ I, int n, long long blk, int last,
                                          double* isg, int* __restrict__ status) {
   const BatchInst& in = I[find_instance(I, n, blk)];
@@ -87,16 +89,16 @@ __device__ __forceinline__ void boe_tile(const BatchInst* __restrict__ I, int n,
   double* out = last ? in.u : in.b;
   oe_inv_sigma<Fields<SYS>::F>(in.sigma, mesh, isg);
   const int form = oe_form(in.g);  // as the single-mesh launch
-  if (form == OE_SQUARE) oe_warp2d<SYS, BC, 0, OE_SQUARE, LD>(in.g, in.a, out, in.dt, isg, status, mesh, i0, j);
+  if (SQUARE || form == OE_SQUARE) oe_warp2d<SYS, BC, 0, OE_SQUARE, LD>(in.g, in.a, out, in.dt, isg, status, mesh, i0, j);
   else if (form == OE_MILD) oe_warp2d<SYS, BC, 0, OE_MILD, LD>(in.g, in.a, out, in.dt, isg, status, mesh, i0, j);
   else oe_warp2d<SYS, BC, 0, OE_OBLONG, LD>(in.g, in.a, out, in.dt, isg, status, mesh, i0, j);
 }
 
-template <int SYS, int BC, int R>
+template <int SYS, int BC, int R, bool SQUARE>
 __global__ void __launch_bounds__(32 * R, 16 / R) k_boe(const BatchInst* __restrict__ I, int n, int last,
                                                         int* __restrict__ status) {
   __shared__ double isg[Fields<SYS>::F];
-  boe_tile<SYS, BC, R, LD_NC>(I, n, blockIdx.x, last, isg, status);
+  boe_tile<SYS, BC, R, LD_NC, SQUARE>(I, n, blockIdx.x, last, isg, status);
 }
 
 // avg and sigma per instance, mesh and field: grid (F, 2, n), one warp each,
@@ -224,7 +226,7 @@ __global__ void __launch_bounds__(32 * R) k_bpersist(BPersistArgs a) {
       if (!grid_sync(a.bar, a.expected, a.status, a.limit_ns)) return;
       for (long long b = blockIdx.x; b < a.ntiles; b += gridDim.x) {
         __syncthreads();  // the previous tile's readers of isg are done
-        boe_tile<SYS, BC, R, LD_CA>(a.I, a.n, b, l == 2, isg, a.status);
+        boe_tile<SYS, BC, R, LD_CA, false>(a.I, a.n, b, l == 2, isg, a.status);
       }
       if (!grid_sync(a.bar, a.expected, a.status, a.limit_ns)) return;
     }
@@ -323,13 +325,13 @@ static cudaError_t launch_bstage_t(cdg_batch* B, int l, double ca, double cb) {
   }
 }
 
-template <int SYS, int BC>
+template <int SYS, int BC, bool SQUARE>
 static cudaError_t launch_boe_t(cdg_batch* B, int last) {
   const unsigned grid = (unsigned)B->total_blocks;
   switch (B->rows) {
-    case 2: k_boe<SYS, BC, 2><<<grid, 64, 0, B->stream>>>(B->d_inst, B->n, last, B->status); break;
-    case 8: k_boe<SYS, BC, 8><<<grid, 256, 0, B->stream>>>(B->d_inst, B->n, last, B->status); break;
-    default: k_boe<SYS, BC, 4><<<grid, 128, 0, B->stream>>>(B->d_inst, B->n, last, B->status); break;
+    case 2: k_boe<SYS, BC, 2, SQUARE><<<grid, 64, 0, B->stream>>>(B->d_inst, B->n, last, B->status); break;
+    case 8: k_boe<SYS, BC, 8, SQUARE><<<grid, 256, 0, B->stream>>>(B->d_inst, B->n, last, B->status); break;
+    default: k_boe<SYS, BC, 4, SQUARE><<<grid, 128, 0, B->stream>>>(B->d_inst, B->n, last, B->status); break;
   }
   return cudaGetLastError();
 }
@@ -342,8 +344,13 @@ static cudaError_t launch_bstage(cdg_batch* B, int l, double ca, double cb) {
 
 static cudaError_t launch_boe(cdg_batch* B, int last) {
   B->launches += 1;
-  if (B->bc == BC_PERIODIC) return launch_boe_t<SYS_EULER, BC_PERIODIC>(B, last);
-  return launch_boe_t<SYS_EULER, BC_TRANSMISSIVE>(B, last);
+  bool square = true;
+  for (int q = 0; q < B->n; ++q) square = square && oe_form(B->h_inst[q].g) == OE_SQUARE;
+  if (B->bc == BC_PERIODIC)
+    return square ? launch_boe_t<SYS_EULER, BC_PERIODIC, true>(B, last)
+                  : launch_boe_t<SYS_EULER, BC_PERIODIC, false>(B, last);
+  return square ? launch_boe_t<SYS_EULER, BC_TRANSMISSIVE, true>(B, last)
+                : launch_boe_t<SYS_EULER, BC_TRANSMISSIVE, false>(B, last);
 }
 
 static const double BSSP3_C[3] = {0.0, 0.75, 1.0 / 3.0};
