@@ -44,11 +44,12 @@ WARP_INST_PEAK = 152 * 4 * 2.07e9 / 1e12
 HBM_FALLBACK_GBS = 6800.0
 
 # Executed warp instructions per cell (one primal or dual cell, 2D Euler Q^2) of
-# the two hot kernels: ncu smsp__inst_executed.sum of one launch at 256^2
-# (periodic, square cells) divided by its cells.
-INST_PER_CELL = {"stage": 1379, "oe": 1040}
-# DRAM bytes per cell per launch from a capture of these kernels: none yet.
-TRAFFIC_PER_CELL = {"stage": None, "oe": None}
+# the two hot kernels: ncu smsp__inst_executed.sum of a launch on the workload's
+# data at 512^2 (transmissive, after 60 steps) divided by its cells.
+INST_PER_CELL = {"stage": 1392, "oe": 1035}
+# DRAM bytes per cell and launch (read + written) from the same capture; the
+# stage's is the mean of a step's three.
+TRAFFIC_PER_CELL = {"stage": 715, "oe": 501}
 # Algorithmic HBM bytes per cell: stage reads u_in (36 doubles) and, in two of
 # three stages, u^n (36), writes u_h (36); OE reads u_h (36), writes u_sigma (36)
 # (neighbour re-reads, of both meshes, are L2 hits: the two meshes' blocks of a
@@ -363,7 +364,7 @@ def run_generic(args, ws, rank, local):
     kms, kcount = prof[kname]
     avg_s = (kms / max(kcount, 1)) * 1e-3
     tiled = k == 2 and args.basis == "Q" and w.rk != 4  # served by the tiled Q^2 kernels
-    ipc = INST_PER_CELL[kname] if tiled else None  # of the degree-generic kernels: no capture yet
+    ipc = INST_PER_CELL[kname] if tiled else None  # counted for the tiled kernels
     roof = {"bound": "alu", "kernel": f"k_{kname}{'2d' if tiled else '2k'} (Euler, periodic, {args.basis}{k})",
             "unit": "T warp instructions/s",
             "peak": WARP_INST_PEAK, "peak_source": "derived: 152 SMs x 4 warp instructions/clk x 2.07 GHz",

@@ -18,8 +18,9 @@ constexpr int NTK = 128;  // threads of an OE block: 4 rows of 8 cells, four lan
 // coefficients as a result (oecdg_oe64.cuh), which write delta in place of the damped state.
 enum { OEK_SQUARE = 0, OEK_OBLONG = 1, OEK_DELTA = 2 };
 //
-// Measured: P^3 Euler 256^2 0.38 ms a launch, P^2 advection
-// 512^2 0.22 ms; the one-thread-per-cell FP64 form took about 2.4 and 1.1 ms.
+// Measured, a launch on square cells: P^3 Euler 256^2 0.34 ms (ALU pipe 60%), P^2 advection
+// 512^2 0.20 ms (FP64 pipe 83%); the one-thread-per-cell FP64 form took about 2.4 and 1.1
+// ms, the FP64 form here 5 times as long as the square one.
 struct OeK {
   double c[2][4];  // [direction][order]: the factor of the integer sums in delta^m
 };
@@ -82,7 +83,6 @@ __global__ void __launch_bounds__(NTK, Modes2<K, B>::M > 10 ? 2 : (K > 2 ? 3 : 4
           if (f == fq) T[n][m] = __double_as_longlong(t);
         }
     } else if constexpr (FORM == OEK_OBLONG) {
-      const bool swap = g.hx < g.hy;
       fx s[2][K + 1];
       int E[K + 1];
       oek_oblong<K, B, LD_NC>(g, us + (long long)(f * M) * P, uo + (long long)(f * M) * P, sx, sy, mx, my, neg, s, E);
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(NTK, Modes2<K, B>::M > 10 ? 2 : (K > 2 ? 3 : 4
       for (int m = 0; m <= K; ++m) {
 #pragma unroll
         for (int n = 0; n < 2; ++n) {
-          fx t = swap ? s[1 - n][m] : s[n][m];
+          fx t = s[n][m];
           t += shfl_xor_fx(t, 8);
           t += shfl_xor_fx(t, 16);
           if (f == fq) T[n][m] = t;
@@ -158,8 +158,13 @@ __global__ void __launch_bounds__(NTK, Modes2<K, B>::M > 10 ? 2 : (K > 2 ? 3 : 4
     // the sums' unit: 2^(ev - 1023 - OEK_FX)
     const double pw = FORM == OEK_DELTA ? 1.0 / oe_unit(isg[fq]) : __hiloint2double((ev[m] - OEK_FX) << 20, 0);
     const double w = ev[0] >= FX_EXNAN ? __longlong_as_double(0x7ff8000000000000LL) : isg[fq] * pw;
-    const double tx = FORM == OEK_DELTA ? __longlong_as_double(T[0][m]) : __ll2double_rn(T[0][m]);
-    const double ty = FORM == OEK_DELTA ? __longlong_as_double(T[1][m]) : __ll2double_rn(T[1][m]);
+    double tx = FORM == OEK_DELTA ? __longlong_as_double(T[0][m]) : __ll2double_rn(T[0][m]);
+    double ty = FORM == OEK_DELTA ? __longlong_as_double(T[1][m]) : __ll2double_rn(T[1][m]);
+    if (FORM == OEK_OBLONG && g.hx < g.hy) {  // read transposed
+      const double t = tx;
+      tx = ty;
+      ty = t;
+    }
     long long key = oe_key(fma(bx * oec.c[0][m], tx, (by * oec.c[1][m]) * ty) * w);
     if (F == 4) {
       key = max(key, shfl_xor_fx(key, 8));

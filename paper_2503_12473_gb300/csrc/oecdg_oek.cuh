@@ -167,7 +167,7 @@ __device__ __forceinline__ void oek_half_face(const fx (&kc)[Modes2<K, B>::M], c
 // are read transposed, and S[0], S[1] are then the half-faces normal to y and x.
 // S[d][m]: the rule's sums in units of 2^(E[m] - 1023 - OEK_FX) 2^m / h_min^m.
 // Measured, a launch of the OE step against that with one exponent: P^3 256 x 250 0.42 ->
-// 0.40 ms, P^2 512 x 500 0.57 -> 0.51 ms, Q^3 256 x 250 0.67 -> 0.78 ms (more registers).
+// 0.40 ms, P^2 512 x 500 0.56 -> 0.51 ms, Q^3 256 x 250 0.67 -> 0.77 ms (its 255 registers).
 template <int K, int B, int LD>
 __device__ __forceinline__ void oek_oblong(const Geo& g, const double* __restrict__ us, const double* __restrict__ uo,
                                            int sx, int sy, int mx, int my, int neg, fx (&S)[2][K + 1],
@@ -186,9 +186,14 @@ __device__ __forceinline__ void oek_oblong(const Geo& g, const double* __restric
     my = t;
   }
   double k[M], o[M];
+  // transposed, Q^k's modes (a, b) lie at a (K+1) + b, P^k's of a total degree in reverse
+  const long long da = B == BASIS_P ? 0 : (swap ? (K + 1) * P : P);
+  const long long db = B == BASIS_P ? (swap ? -P : P) : (swap ? P : (K + 1) * P);
 #pragma unroll
   for (int m = 0; m < M; ++m) {
-    const long long at = (swap ? oek_mode<K, B, 1>(MD::a(m), MD::b(m)) : m) * P;
+    const int s = MD::a(m) + MD::b(m);
+    const long long row = B == BASIS_Q ? 0 : (s * (s + 1) / 2 + (swap ? s : 0)) * P;
+    const long long at = row + MD::a(m) * da + MD::b(m) * db;
     k[m] = ldv<LD>(us + at);
     o[m] = ldv<LD>(uo + at);
   }
