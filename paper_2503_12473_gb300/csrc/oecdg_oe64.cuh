@@ -5,7 +5,9 @@
 // cell's local variation: enough for the decay, since sigma is at least that variation's
 // size, but a coefficient by itself can be far below it (third derivatives of smooth data:
 // P^3 on a wave over 128 cells has delta^3 to 1e-11 from the fixed-point sums, to 2e-16
-// from these, at about 5 times the time).
+// from these).  The FP64 pipe sets their time, as it did the OE step's before the
+// fixed-point sums: a launch takes 2.30 ms on P^3 Euler 256^2 (2.4 there) where the step takes
+// 0.34, 6.1 on Q^2 512^2 (0.62).
 #pragma once
 
 #include "oecdg_common.cuh"
@@ -79,30 +81,36 @@ static __device__ __noinline__ void oe_quarter_fp64(const double* __restrict__ u
         E[d][a] = e;
       }
     const double sn = n == 0 ? rx : ry, st = n == 0 ? ry : rx;
+    double pn = 1.0, pt[K + 1];
+    pt[0] = 1.0;
+#pragma unroll
+    for (int d = 1; d <= K; ++d) {
+      pn *= sn;
+      pt[d] = pt[d - 1] * st;
+#pragma unroll
+      for (int a = 0; a <= K; ++a) E[d][a] *= pn;
+    }
     double s[K + 1];
 #pragma unroll
     for (int m = 0; m <= K; ++m) s[m] = 0.0;
-#pragma unroll 1
+#pragma unroll
     for (int q = 0; q < N; ++q) {
-      const double wq = GWK[N - 2][q], t = 0.5 * GNK[N - 2][q] - 0.5;
+      const double wq = gw1(N, q), t = 0.5 * gn1(N, q) - 0.5;
 #pragma unroll
       for (int m = 0; m <= K; ++m) {
         double ss = 0.0;
 #pragma unroll
         for (int an = 0; an <= m; ++an) {
           const int at = m - an;
-          double v = 0.0, sc = 1.0;
+          double v = 0.0;
 #pragma unroll
           for (int a = at; a <= K; ++a)
             if (!(B == BASIS_P && a + an > K)) v = fma(E[an][a], lpd(a, at, t), v);
-#pragma unroll
-          for (int r = 0; r < an; ++r) sc *= sn;
-#pragma unroll
-          for (int r = 0; r < at; ++r) sc *= st;
-          v *= sc;
+          if (at > 0) v *= pt[at];
           ss = fma(v, v, ss);
         }
-        s[m] = fma(wq, sqrt(ss), s[m]);
+        // sums below 2^-1022 are far below the unit
+        if (__double2hiint(ss) >= 0x00100000) s[m] = fma(wq, sqrt_pos(ss), s[m]);
       }
     }
 #pragma unroll
