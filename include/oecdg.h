@@ -187,7 +187,9 @@ cdg_status cdg_rk_combine(cdg_ctx* ctx, const double* d_ul, int n, const double*
 cdg_status cdg_oe_damp(cdg_ctx* ctx, const double* d_uh, double* d_usig);
 
 /* The damping coefficients alone, for inspection: d_delta [2][nys][nxs][k+1]
- * (the padded layout), d_sigma [2][fields] (either may be NULL). */
+ * (the padded layout), d_sigma [2][fields] (either may be NULL).  2D: from sums
+ * in FP64, each delta_K^m to its own rounding, at several times the cost of the OE
+ * step, whose sums are cut relative to the cell's variation. */
 cdg_status cdg_oe_coefficients(cdg_ctx* ctx, const double* d_uh, double* d_delta, double* d_sigma);
 
 /* nsteps full time steps of Eq. (eq:RKCDG) in place on d_u, starting at time t

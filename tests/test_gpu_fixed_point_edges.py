@@ -330,3 +330,45 @@ def test_a_tuning_file_of_other_kernels_is_not_used(tmp_path):
     new = json.loads(path.read_text())
     assert len(new) == 2 and new.pop(next(iter(old))) == 801
     assert list(new.values()) == [100 * rows + b.cdg_batch_grid()[0]]
+
+
+@pytest.mark.parametrize("bx,by", [(6.0, 1.0), (1.0, 3.0)])
+@pytest.mark.parametrize("sides", sorted(SIDES))
+@pytest.mark.parametrize("system", [O.EULER, O.ADVECTION])
+@pytest.mark.parametrize("k,basis", [(2, O.BASIS_Q), (3, O.BASIS_P)])
+def test_steps_on_oblong_cells(k, basis, system, sides, bx, by):
+    """Damping and two steps at aspect ratios of 3 to 6 either way, every side
+    condition: 1e-12 relative L1, as elsewhere for two steps of smooth data."""
+    if sides == "walls" and system != O.EULER:
+        pytest.skip("walls need the Euler equations")
+    p, ctx = _pair(system, k, basis, 13, 12, bx=bx, by=by, bc=SIDES[sides], rk=k + 1)
+    u = _state(p, np.random.default_rng(7))
+    ug = torch.from_numpy(u).cuda()
+    out = torch.zeros_like(ug)
+    ctx.cdg_set_dt(0.7e-3, 1e-3)
+    ctx.cdg_oe_damp(ug, out)
+    ref, st = O.oe(p, u, 0.7e-3)
+    assert st == O.OK and np.abs(out.cpu().numpy() - ref).sum() <= 1e-12 * np.abs(ref).sum()
+    ctx.cdg_step(ug, 0.0, 0.0, 2)
+    ref, _, n, st = O.advance(p, u, 0.0, 0.0, 2)
+    assert st == O.OK and n == 2 and np.abs(ug.cpu().numpy() - ref).sum() <= 1e-12 * np.abs(ref).sum()
+
+
+@pytest.mark.parametrize("bx,by", [(10.0, 1.0), (1.0, 6.0)])
+@pytest.mark.parametrize("system,nx,ny", [(O.ADVECTION, 6, 5), (O.EULER, 4, 3)])
+def test_adjoint_on_oblong_cells(system, nx, ny, bx, by):
+    """J^T lam of a step with the OE step's recorded sums on cells of aspect ratio 4 to 8
+    against the oracle's own adjoint (complex step), with the bars of square cells."""
+    p, ctx = _pair(system, 2, O.BASIS_Q, nx, ny, bx=bx, by=by)
+    rng = np.random.default_rng(4)
+    u = 0.05 * rng.uniform(-1.0, 1.0, p.shape)
+    if system == O.EULER:
+        u[:, 0, 0] += 1.0
+        u[:, 3, 0] += 2.5
+    lam = rng.uniform(-1.0, 1.0, p.shape)
+    ref, st = O.step_adjoint(p, u, lam)
+    assert st == O.OK
+    got = torch.empty(p.shape, dtype=torch.float64, device="cuda")
+    ctx.cdg_step_adjoint(torch.from_numpy(u).cuda(), torch.from_numpy(lam).cuda(), got)
+    err = np.abs(got.cpu().numpy() - ref)
+    assert err.sum() <= 1e-10 * np.abs(ref).sum() and err.max() <= 1e-9 * np.abs(ref).max()
